@@ -403,10 +403,11 @@ class VTRender(torch.autograd.Function):
     must hold their current values (call scene.update after changing them)."""
 
     @staticmethod
-    def forward(ctx, sites, sigma, tex, tex_vd, o, d, scene, params, with_dist=False):
+    def forward(ctx, sites, sigma, tex, tex_vd, o, d, scene, params, with_dist=False, grad_mode=True):
         res = torch.empty(o.shape[0], 3, device=o.device)
         dist = torch.empty(o.shape[0], 3, device=o.device) if with_dist else None
-        rec = walk_record(o.shape[0], o.device) if any(ctx.needs_input_grad[:4]) else None
+        # (the mode of the caller: it is off in here, and needs_input_grad does not look at it)
+        rec = walk_record(o.shape[0], o.device) if grad_mode and any(ctx.needs_input_grad[:4]) else None
         rgb = torch.empty(o.shape[0], 3, device=o.device)
         render_fwd(scene, o, d, params, out=(rgb, None, None), residual=res, dist=dist, record=rec)
         ctx.scene, ctx.params, ctx.with_dist = scene, params, with_dist
@@ -425,13 +426,10 @@ class VTRender(torch.autograd.Function):
         gs, gsig, gt = render_bwd(ctx.scene, o, d, ctx.params, rgb, grad_rgb, need=need, residual=res,
                                   tex_vd_out=gvd, dist=dist, grad_dist=grad_dist if ctx.with_dist else None,
                                   record=rec)
-        return gs, gsig, gt, gvd, None, None, None, None, None
+        return gs, gsig, gt, gvd, None, None, None, None, None, None
 
 
 def render(sites, sigma, tex, o, d, scene: Scene, params, tex_vd=None, with_dist=False):
     """Differentiable render; returns rgb, or (rgb, L_dist per ray) with
     with_dist=True (distortion loss of Sec. 5.3, Eq. 2)."""
-    if not torch.is_grad_enabled():  # no backward will come: no record of the walk
-        sites, sigma, tex, tex_vd = (x.detach() if isinstance(x, torch.Tensor) else x
-                                     for x in (sites, sigma, tex, tex_vd))
-    return VTRender.apply(sites, sigma, tex, tex_vd, o, d, scene, params, with_dist)
+    return VTRender.apply(sites, sigma, tex, tex_vd, o, d, scene, params, with_dist, torch.is_grad_enabled())
