@@ -127,11 +127,9 @@ class Trainer:
         self.record = api.walk_record(B, self.dev)  # the step's walk, from its forward to its backward
         self.grad_rgb = torch.empty(B, 3, device=self.dev)
         self.gdist = torch.full((B,), cfg.lambda_dist / B, device=self.dev)
-        # the samples' launch layout, unless the caller's parameters give one
-        laid_out = render_params.get("img_w") or render_params.get("image_sizes") is not None
-        tiles = None if laid_out else sample_tiles(cams, B)
-        self.step_params = self.rparams if tiles is None else api.make_params(**render_params, appearance=1,
-                                                                              image_sizes=tiles)
+        # the samples' launch layout, for parameters that have none
+        tiles = sample_tiles(cams, B)
+        self.tiles = None if tiles is None else api.make_params(image_sizes=tiles)
         self.loss = torch.empty(1, device=self.dev)
         self.reg = torch.empty(1, device=self.dev)
         n, R = self.p["tex"].shape[0], self.p["tex"].shape[1]
@@ -164,9 +162,19 @@ class Trainer:
         self.refreshes += 1
 
     # ------------------------------------------------------------------ one iteration
+    def step_params(self):
+        """The render parameters as they stand, with the samples' launch layout unless they have their own."""
+        p, t = self.rparams, self.tiles
+        if t is None or p.img_w > 0 or p.image_sizes:
+            return p
+        p = type(p).from_buffer_copy(p)
+        p.image_sizes, p.n_images = t.image_sizes, t.n_images
+        return p
+
     def step(self, sync_loss=False):
         cfg, s = self.cfg, _vt
         st = api._stream()
+        params = self.step_params()
         if self.it > 0 and cfg.refresh_every > 0 and self.it % cfg.refresh_every == 0:
             self.refresh()
         _vt.vt_sigma_from_rho(self.sigma.numel(), self.p["rho"].data_ptr(), self.sigma.data_ptr(), st)
@@ -174,16 +182,16 @@ class Trainer:
         s.vt_sample_rays(self.n_pool, self.o_pool.data_ptr(), self.d_pool.data_ptr(), self.y_pool.data_ptr(), self.B,
                          cfg.seed * 1_000_003 + self.it, self.o.data_ptr(), self.d.data_ptr(), self.y.data_ptr(),
                          0, st)
-        api.render_fwd(self.scene, self.o, self.d, self.step_params, out=(self.rgb, None, None), residual=self.res,
+        api.render_fwd(self.scene, self.o, self.d, params, out=(self.rgb, None, None), residual=self.res,
                        dist=self.dist, record=self.record)
         s.vt_smooth_l1_loss(self.B, self.rgb.data_ptr(), self.y.data_ptr(), cfg.smooth_l1_beta,
                             self.grad_rgb.data_ptr(), self.loss.data_ptr(), st)
         if cfg.scene_order_grads:
-            self._fused_update(st)
+            self._fused_update(st, params)
             if sync_loss:
                 return self.loss.item(), self.reg.item(), self.dist[:, 0].mean().item()
             return None
-        api.render_bwd(self.scene, self.o, self.d, self.step_params, self.rgb, self.grad_rgb,
+        api.render_bwd(self.scene, self.o, self.d, params, self.rgb, self.grad_rgb,
                        out=(self.g["sites"], self.gsig, self.g["tex"]), residual=self.res, dist=self.dist,
                        grad_dist=self.gdist, tex_vd_out=self.g["tex_vd"], record=self.record)
         n = self.p["tex"].shape[0]
@@ -202,12 +210,12 @@ class Trainer:
             return self.loss.item(), self.reg.item(), self.dist[:, 0].mean().item()
         return None
 
-    def _fused_update(self, st):
+    def _fused_update(self, st, params):
         """Backward with the gradients left in scene order, then one fused Adam
         step per texture map (with its regulariser) and one for sites and
         densities (with Eq. 4): no user-order gradient arrays are written."""
         cfg, s = self.cfg, _vt
-        gc, gt, gv = api.render_bwd_scene_order(self.scene, self.o, self.d, self.step_params, self.rgb, self.grad_rgb,
+        gc, gt, gv = api.render_bwd_scene_order(self.scene, self.o, self.d, params, self.rgb, self.grad_rgb,
                                                 residual=self.res, dist=self.dist, grad_dist=self.gdist,
                                                 record=self.record)
         lrs = learning_rates(cfg, self.it)
