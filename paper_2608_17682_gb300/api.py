@@ -408,24 +408,27 @@ class VTRender(torch.autograd.Function):
         dist = torch.empty(o.shape[0], 3, device=o.device) if with_dist else None
         # (the mode of the caller: it is off in here, and needs_input_grad does not look at it)
         rec = walk_record(o.shape[0], o.device) if grad_mode and any(ctx.needs_input_grad[:4]) else None
+        # The record lives and dies with the saved residual, but is not itself a saved tensor: hooks that pack those
+        # (offloading, checkpointing) would move ten times the bytes for what the backward can do without.
+        res.walk = rec
         rgb = torch.empty(o.shape[0], 3, device=o.device)
         render_fwd(scene, o, d, params, out=(rgb, None, None), residual=res, dist=dist, record=rec)
         ctx.scene, ctx.params, ctx.with_dist = scene, params, with_dist
-        ctx.save_for_backward(o, d, rgb, res, dist, rec)
+        ctx.save_for_backward(o, d, rgb, res, dist)
         if with_dist:
             return rgb, dist[:, 0].contiguous()
         return rgb
 
     @staticmethod
     def backward(ctx, grad_rgb, grad_dist=None):
-        o, d, rgb, res, dist, rec = ctx.saved_tensors
+        o, d, rgb, res, dist = ctx.saved_tensors
         need = ctx.needs_input_grad[:3]
         gvd = None
         if ctx.needs_input_grad[3] and ctx.scene.has_tex_vd:
             gvd = torch.empty(ctx.scene.n, ctx.scene.R, ctx.scene.R, 3, device=o.device)
         gs, gsig, gt = render_bwd(ctx.scene, o, d, ctx.params, rgb, grad_rgb, need=need, residual=res,
                                   tex_vd_out=gvd, dist=dist, grad_dist=grad_dist if ctx.with_dist else None,
-                                  record=rec)
+                                  record=getattr(res, "walk", None))
         return gs, gsig, gt, gvd, None, None, None, None, None, None
 
 

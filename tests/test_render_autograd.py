@@ -1,4 +1,6 @@
 """The autograd entry point without a GPU, its kernel calls replaced: what it refuses and what it records."""
+import weakref
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -13,14 +15,22 @@ class StandIn:
 
 @pytest.fixture
 def calls(monkeypatch):
-    """Records of the forward calls; colours are zero."""
+    """Records (as weak references) that the forward and backward calls got; colours and gradients are zero."""
     made = []
 
+    def note(record):
+        made.append(None if record is None else weakref.ref(record))
+
     def render_fwd(scene, o, d, params, out=None, record=None, **kw):
-        made.append(record)
+        note(record)
         out[0].zero_()
 
+    def render_bwd(scene, *a, record=None, **kw):
+        note(record)
+        return torch.zeros(4, 3), torch.zeros(4), torch.zeros(4, 2, 2, 3)
+
     monkeypatch.setattr(api, "render_fwd", render_fwd)
+    monkeypatch.setattr(api, "render_bwd", render_bwd)
     return made
 
 
@@ -37,7 +47,7 @@ def test_a_tangent_is_refused(calls, grad_mode, which):
     with fwad.dual_level(), torch.set_grad_enabled(grad_mode):
         x[which] = fwad.make_dual(x[which], torch.ones_like(x[which]))
         with pytest.raises((NotImplementedError, RuntimeError)):
-            api.render(*x, o, d, StandIn(), None)
+            api.render(*x, o, d, StandIn(), api.make_params())
 
 
 @pytest.mark.parametrize("grad_mode", [True, False])
@@ -46,6 +56,33 @@ def test_a_walk_is_recorded_only_for_a_backward(calls, grad_mode, needs):
     sites, sigma, tex, o, d = arrays()
     sigma.requires_grad_(needs)
     with torch.set_grad_enabled(grad_mode):
-        rgb = api.render(sites, sigma, tex, o, d, StandIn(), None)
+        rgb = api.render(sites, sigma, tex, o, d, StandIn(), api.make_params())
     assert rgb.requires_grad == (grad_mode and needs)
     assert (calls[0] is not None) == (grad_mode and needs)
+
+
+def render(needs_grad=True):
+    sites, sigma, tex, o, d = arrays()
+    return api.render(sites, sigma.requires_grad_(needs_grad), tex, o, d, StandIn(), api.make_params())
+
+
+def test_the_record_lives_as_long_as_the_saved_tensors(calls):
+    rgb = render()
+    rgb.sum().backward(retain_graph=True)
+    rgb.sum().backward()
+    assert calls[0] is calls[1] is calls[2]
+    assert calls[0]() is None  # rgb and its node are still here
+
+
+def test_hooks_of_saved_tensors_do_not_see_the_record(calls):
+    packed = []
+
+    def pack(t):
+        packed.append(t.nbytes)
+        return t.clone()
+
+    with torch.autograd.graph.saved_tensors_hooks(pack, lambda t: t):
+        rgb = render()
+    assert sorted(packed) == [16 * 3 * 4] * 4  # o, d, rgb, residual
+    rgb.sum().backward()
+    assert calls[1] is None  # the residual that came back is another tensor: the backward searches
