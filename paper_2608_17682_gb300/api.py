@@ -8,7 +8,10 @@ follows the record and searches only the steps that it does not hold.
 """
 from __future__ import annotations
 
+import collections
 import ctypes
+import threading
+import weakref
 
 import torch
 
@@ -88,7 +91,7 @@ class Scene:
                                  (_vt.VT_SCENE_KEEP_ORDER if keep_order else 0)
                                  | (_vt.VT_SCENE_HALF_OFFSETS if half_offsets else 0), _ptr(tvd))
         with torch.cuda.device(device):
-            self.handle = _vt.vt_scene_create(desc, _stream())
+            self.handle = with_room(lambda: _vt.vt_scene_create(desc, _stream()))
         self.n_edges = _vt.vt_scene_info(self.handle)[3]
 
     @classmethod
@@ -181,23 +184,71 @@ def generate_rays(cameras, device="cuda", out=None):
 
 
 # A walk record holds up to RECORD_STEPS steps of every ray (the rays of the
-# surface scenes take 7 to 19 cells on average, 60 at most), fewer where it
-# would pass RECORD_BYTES; what it does not hold is searched again.
+# surface scenes take 7 to 19 cells on average, 60 at most), fewer where the
+# records alive on a device would pass RECORD_BYTES together; what a record does
+# not hold is searched again.
 RECORD_STEPS = 48
 RECORD_BYTES = 1 << 30
 
 
-def walk_record(n, device):
+def walk_record(n, device, held=0):
     """Memory for render_fwd(record=) of n rays: int64 [steps + 2, n] (8 bytes
-    per step, opaque), or None where it would hold less than 8 steps or the
-    device has no room for it."""
-    steps = min(RECORD_STEPS, RECORD_BYTES // (8 * n) - 2) if n else 0
+    per step, opaque), or None where it would hold less than 8 steps within
+    RECORD_BYTES less `held` bytes, or the device has no room for it."""
+    steps = min(RECORD_STEPS, (RECORD_BYTES - held) // (8 * n) - 2) if n else 0
     if steps < 8:
         return None
     try:
         return torch.empty(steps + 2, n, dtype=torch.int64, device=device)
     except torch.cuda.OutOfMemoryError:
         return None
+
+
+class Walk:
+    """A walk record (`record`, None without one) that counts towards RECORD_BYTES
+    of its device while it lives, and that with_room may take back."""
+
+    _lock = threading.RLock()  # reentrant: a collection within it may end another's life
+    _alive = weakref.WeakSet()
+    _held = collections.Counter()  # bytes per device
+
+    def __init__(self, n, device):
+        self.record, device = None, torch.device(device)
+        if device.type == "cuda" and device.index is None:
+            device = torch.device("cuda", torch.cuda.current_device())
+        self._device = device
+        with self._lock:
+            self.record = walk_record(n, device, self._held[device])
+            if self.record is not None:
+                self._held[device] += self.record.nbytes
+                self._alive.add(self)
+
+    def give_up(self):
+        with self._lock:
+            if self.record is not None:
+                self._held[self._device] -= self.record.nbytes
+                self.record = None
+
+    __del__ = give_up
+
+
+def with_room(call):
+    """call(), and, where the device's memory does not suffice for it, again
+    without any walk record: they only save time."""
+    try:
+        return call()
+    except (torch.cuda.OutOfMemoryError, VTError) as e:
+        if isinstance(e, VTError) and e.status != _vt.VT_ERR_OOM:
+            raise
+        with Walk._lock:
+            walks = [w for w in Walk._alive if w.record is not None]
+        if not walks:
+            raise
+    # (outside the handler, whose exception holds on to the failed call's locals)
+    for w in walks:
+        w.give_up()
+    torch.cuda.empty_cache()  # to the driver: the library allocates there
+    return call()
 
 
 def _record_steps(record, n):
@@ -395,6 +446,12 @@ def average_samples_bwd(grad_px, spp):
     return out
 
 
+def _walk_of(res):
+    """The walk record that a saved residual carries, if any."""
+    walk = getattr(res, "walk", None)
+    return None if walk is None else walk.record
+
+
 class VTRender(torch.autograd.Function):
     """Differentiable render of rays (o, d) through a Scene.
 
@@ -406,13 +463,13 @@ class VTRender(torch.autograd.Function):
     def forward(ctx, sites, sigma, tex, tex_vd, o, d, scene, params, with_dist=False, grad_mode=True):
         res = torch.empty(o.shape[0], 3, device=o.device)
         dist = torch.empty(o.shape[0], 3, device=o.device) if with_dist else None
-        # (the mode of the caller: it is off in here, and needs_input_grad does not look at it)
-        rec = walk_record(o.shape[0], o.device) if grad_mode and any(ctx.needs_input_grad[:4]) else None
-        # The record lives and dies with the saved residual, but is not itself a saved tensor: hooks that pack those
-        # (offloading, checkpointing) would move ten times the bytes for what the backward can do without.
-        res.walk = rec
         rgb = torch.empty(o.shape[0], 3, device=o.device)
-        render_fwd(scene, o, d, params, out=(rgb, None, None), residual=res, dist=dist, record=rec)
+        # The record comes last, what the render needs first. It lives and dies with the saved residual, but is not
+        # itself a saved tensor: hooks that pack those (offloading, checkpointing) would move ten times the bytes for
+        # what the backward can do without. (grad_mode: it is off in here, and needs_input_grad does not look at it.)
+        if grad_mode and any(ctx.needs_input_grad[:4]):
+            res.walk = Walk(o.shape[0], o.device)
+        render_fwd(scene, o, d, params, out=(rgb, None, None), residual=res, dist=dist, record=_walk_of(res))
         ctx.scene, ctx.params, ctx.with_dist = scene, params, with_dist
         ctx.save_for_backward(o, d, rgb, res, dist)
         if with_dist:
@@ -423,12 +480,15 @@ class VTRender(torch.autograd.Function):
     def backward(ctx, grad_rgb, grad_dist=None):
         o, d, rgb, res, dist = ctx.saved_tensors
         need = ctx.needs_input_grad[:3]
-        gvd = None
-        if ctx.needs_input_grad[3] and ctx.scene.has_tex_vd:
-            gvd = torch.empty(ctx.scene.n, ctx.scene.R, ctx.scene.R, 3, device=o.device)
-        gs, gsig, gt = render_bwd(ctx.scene, o, d, ctx.params, rgb, grad_rgb, need=need, residual=res,
-                                  tex_vd_out=gvd, dist=dist, grad_dist=grad_dist if ctx.with_dist else None,
-                                  record=getattr(res, "walk", None))
+
+        def gradients():
+            gvd = None
+            if ctx.needs_input_grad[3] and ctx.scene.has_tex_vd:
+                gvd = torch.empty(ctx.scene.n, ctx.scene.R, ctx.scene.R, 3, device=o.device)
+            return *render_bwd(ctx.scene, o, d, ctx.params, rgb, grad_rgb, need=need, residual=res, tex_vd_out=gvd,
+                               dist=dist, grad_dist=grad_dist if ctx.with_dist else None, record=_walk_of(res)), gvd
+
+        gs, gsig, gt, gvd = with_room(gradients)
         return gs, gsig, gt, gvd, None, None, None, None, None, None
 
 

@@ -124,7 +124,6 @@ class Trainer:
         self.rgb = torch.empty(B, 3, device=self.dev)
         self.res = torch.empty(B, 3, device=self.dev)
         self.dist = torch.empty(B, 3, device=self.dev)
-        self.record = api.walk_record(B, self.dev)  # the step's walk, from its forward to its backward
         self.grad_rgb = torch.empty(B, 3, device=self.dev)
         self.gdist = torch.full((B,), cfg.lambda_dist / B, device=self.dev)
         # the samples' launch layout, for parameters that have none
@@ -143,6 +142,7 @@ class Trainer:
         self.refreshes = 0
         self.scene = None
         self._build_scene(offsets, indices)
+        self.walk = api.Walk(B, self.dev)  # the step's walk, from its forward to its backward
 
     # ------------------------------------------------------------------ topology
     def _build_scene(self, offsets=None, indices=None):
@@ -183,7 +183,7 @@ class Trainer:
                          cfg.seed * 1_000_003 + self.it, self.o.data_ptr(), self.d.data_ptr(), self.y.data_ptr(),
                          0, st)
         api.render_fwd(self.scene, self.o, self.d, params, out=(self.rgb, None, None), residual=self.res,
-                       dist=self.dist, record=self.record)
+                       dist=self.dist, record=self.walk.record)
         s.vt_smooth_l1_loss(self.B, self.rgb.data_ptr(), self.y.data_ptr(), cfg.smooth_l1_beta,
                             self.grad_rgb.data_ptr(), self.loss.data_ptr(), st)
         if cfg.scene_order_grads:
@@ -191,9 +191,10 @@ class Trainer:
             if sync_loss:
                 return self.loss.item(), self.reg.item(), self.dist[:, 0].mean().item()
             return None
-        api.render_bwd(self.scene, self.o, self.d, params, self.rgb, self.grad_rgb,
-                       out=(self.g["sites"], self.gsig, self.g["tex"]), residual=self.res, dist=self.dist,
-                       grad_dist=self.gdist, tex_vd_out=self.g["tex_vd"], record=self.record)
+        api.with_room(lambda: api.render_bwd(
+            self.scene, self.o, self.d, params, self.rgb, self.grad_rgb,
+            out=(self.g["sites"], self.gsig, self.g["tex"]), residual=self.res, dist=self.dist, grad_dist=self.gdist,
+            tex_vd_out=self.g["tex_vd"], record=self.walk.record))
         n = self.p["tex"].shape[0]
         s.vt_texture_regularizers(n, self.R, self.p["tex"].data_ptr(), self.p["tex_vd"].data_ptr(), cfg.lambda_vd,
                                   cfg.lambda_mean, self.g["tex"].data_ptr(), self.g["tex_vd"].data_ptr(),
@@ -215,9 +216,9 @@ class Trainer:
         step per texture map (with its regulariser) and one for sites and
         densities (with Eq. 4): no user-order gradient arrays are written."""
         cfg, s = self.cfg, _vt
-        gc, gt, gv = api.render_bwd_scene_order(self.scene, self.o, self.d, params, self.rgb, self.grad_rgb,
-                                                residual=self.res, dist=self.dist, grad_dist=self.gdist,
-                                                record=self.record)
+        gc, gt, gv = api.with_room(lambda: api.render_bwd_scene_order(
+            self.scene, self.o, self.d, params, self.rgb, self.grad_rgb, residual=self.res, dist=self.dist,
+            grad_dist=self.gdist, record=self.walk.record))
         lrs = learning_rates(cfg, self.it)
         self.it += 1
         n = self.p["tex"].shape[0]

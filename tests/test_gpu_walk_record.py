@@ -88,3 +88,25 @@ def test_record_is_left_out_where_it_does_not_fit():
     assert api.walk_record(0, DEV) is None and api.walk_record(n, "meta") is None
     assert api.walk_record(n - 1, "meta").shape == (10, n - 1)
     assert api.walk_record(100, "meta").shape == (api.RECORD_STEPS + 2, 100)
+
+
+@pytest.mark.parametrize("room", [0, 12, 70, 10_000])
+def test_gradients_do_not_depend_on_the_room_for_records(monkeypatch, room):
+    """Three renders alive before one backward, under bounds that hold some steps of the first record to all of all."""
+    sc = W.make_scene("uniform", 2000, 3, 65)
+    scene = api.Scene.from_workload(sc)
+    rng = np.random.default_rng(66)
+    n = 700
+    P = api.make_params(t_far=2.0)
+    leaves = [torch.as_tensor(x, device=DEV).requires_grad_(True) for x in (sc.sites, sc.sigma, sc.tex)]
+    rays = []
+    for _ in range(3):
+        d = rng.normal(size=(n, 3))
+        rays.append([torch.as_tensor(x.astype(np.float32), device=DEV)
+                     for x in (rng.uniform(0, 1, (n, 3)), d / np.linalg.norm(d, axis=1, keepdims=True))])
+    monkeypatch.setattr(api, "RECORD_BYTES", 0)
+    want = [sum(g) for g in zip(*(torch.autograd.grad(api.render(*leaves, o, d, scene, P).square().sum(), leaves)
+                                  for o, d in rays))]
+    monkeypatch.setattr(api, "RECORD_BYTES", 8 * n * room)
+    got = torch.autograd.grad(sum(api.render(*leaves, o, d, scene, P).square().sum() for o, d in rays), leaves)
+    assert all(close(a, b) for a, b in zip(got, want))

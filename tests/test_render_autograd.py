@@ -86,3 +86,60 @@ def test_hooks_of_saved_tensors_do_not_see_the_record(calls):
     assert sorted(packed) == [16 * 3 * 4] * 4  # o, d, rgb, residual
     rgb.sum().backward()
     assert calls[1] is None  # the residual that came back is another tensor: the backward searches
+
+
+STEP = 8 * 16  # bytes of a step of the stand-in's 16 rays
+
+
+def test_renders_that_live_together_share_the_bound(calls, monkeypatch):
+    monkeypatch.setattr(api, "RECORD_BYTES", STEP * (api.RECORD_STEPS + 2 + 30) + 1)
+    for _ in range(2):  # what the first round held is given back
+        alive = [render() for _ in range(4)]
+        assert [r and r().shape[0] for r in calls] == [api.RECORD_STEPS + 2, 30, None, None]
+        sum(x.sum() for x in alive).backward()
+        del calls[:], alive
+
+
+def fails_with_records(calls, monkeypatch, error):
+    """render_bwd raises while it gets a record, or always where there never was one."""
+    given, plain = [], api.render_bwd
+
+    def render_bwd(*a, record=None, **kw):
+        given.append(record is not None)
+        if record is not None or not calls[0]:
+            raise error()
+        return plain(*a, **kw)
+
+    monkeypatch.setattr(api, "render_bwd", render_bwd)
+    return given
+
+
+def no_room():
+    return api.VTError(api._vt.VT_ERR_OOM)
+
+
+def fault():
+    return api.VTError(api._vt.VT_ERR_CUDA)
+
+
+OOM = [no_room, torch.cuda.OutOfMemoryError]
+
+
+@pytest.mark.parametrize("error", OOM)
+def test_a_backward_without_room_gives_up_the_records(calls, monkeypatch, error):
+    given = fails_with_records(calls, monkeypatch, error)
+    first, second = render(), render()
+    second.sum().backward()
+    first.sum().backward()
+    assert given == [True, False, False]
+    assert calls[0]() is None and calls[1]() is None
+
+
+@pytest.mark.parametrize("error", OOM + [fault])
+def test_other_failures_stay(calls, monkeypatch, error):
+    if error is not fault:
+        monkeypatch.setattr(api, "RECORD_BYTES", 0)  # no records to give up
+    given = fails_with_records(calls, monkeypatch, error)
+    with pytest.raises((api.VTError, torch.cuda.OutOfMemoryError)):
+        render().sum().backward()
+    assert len(given) == 1

@@ -15,7 +15,7 @@ POOL = 2 * 64 * 48
 def trainer(monkeypatch):
     class Scene:
         def __init__(self, *a, **kw):
-            pass
+            assert not any(train.api.Walk._held.values())  # the record comes after the memory that is needed
 
         def permutation(self):
             return None
@@ -46,6 +46,13 @@ def test_the_callers_layout_stays(trainer, rp):
     t = trainer(**rp)
     p = t.step_params()
     assert (p.img_w, p.image_sizes, p.n_images) == (t.rparams.img_w, t.rparams.image_sizes, rp.get("n_images", 1))
+
+
+def test_the_record_counts_while_the_trainer_lives(trainer):
+    t = trainer()
+    assert t.walk.record.nbytes == sum(train.api.Walk._held.values()) > 0
+    del t
+    assert not any(train.api.Walk._held.values())
 
 
 def test_later_changes_reach_the_steps(trainer):
