@@ -85,6 +85,7 @@ class Scene:
                 or tex.shape[1] != tex.shape[2] or tex.shape[3] != 3 or off.shape != (n + 1,):
             raise ValueError("bad scene shapes")
         self.n, self.R = n, tex.shape[1]
+        self.updates = 0
         self.tex_dtype = _DTYPES[tex_dtype] if isinstance(tex_dtype, str) else int(tex_dtype)
         desc = _vt.vt_scene_desc(n, self.R, self.tex_dtype, sites.data_ptr(), sigma.data_ptr(), tex.data_ptr(),
                                  off.data_ptr(), idx.data_ptr(),
@@ -107,6 +108,7 @@ class Scene:
             _arr(x, name, shape, optional=True)
         if keep[3] is not None and not self.has_tex_vd:
             raise ValueError("tex_vd given for a scene built without one")
+        self.updates += 1
         _vt.vt_scene_update(self.handle, *[_ptr(x) for x in keep], _stream())
 
     def permutation(self):
@@ -446,10 +448,16 @@ def average_samples_bwd(grad_px, spp):
     return out
 
 
-def _walk_of(res):
-    """The walk record that a saved residual carries, if any."""
+def _walk_key(scene, params):
+    """What a walk depends on beside its rays: the scene's values and the render parameters (not their timing events)."""
+    return scene.updates, bytes(params)[:_vt.vt_render_params.walk_events.offset]
+
+
+def _walk_of(res, scene, params):
+    """The walk record that a saved residual carries, unless the scene or the parameters have changed since: then the
+    backward walks the scene as it is."""
     walk = getattr(res, "walk", None)
-    return None if walk is None else walk.record
+    return None if walk is None or res.walk_key != _walk_key(scene, params) else walk.record
 
 
 class VTRender(torch.autograd.Function):
@@ -469,7 +477,9 @@ class VTRender(torch.autograd.Function):
         # what the backward can do without. (grad_mode: it is off in here, and needs_input_grad does not look at it.)
         if grad_mode and any(ctx.needs_input_grad[:4]):
             res.walk = Walk(o.shape[0], o.device)
-        render_fwd(scene, o, d, params, out=(rgb, None, None), residual=res, dist=dist, record=_walk_of(res))
+            res.walk_key = _walk_key(scene, params)
+        render_fwd(scene, o, d, params, out=(rgb, None, None), residual=res, dist=dist,
+                   record=_walk_of(res, scene, params))
         ctx.scene, ctx.params, ctx.with_dist = scene, params, with_dist
         ctx.save_for_backward(o, d, rgb, res, dist)
         if with_dist:
@@ -486,7 +496,7 @@ class VTRender(torch.autograd.Function):
             if ctx.needs_input_grad[3] and ctx.scene.has_tex_vd:
                 gvd = torch.empty(ctx.scene.n, ctx.scene.R, ctx.scene.R, 3, device=o.device)
             return *render_bwd(ctx.scene, o, d, ctx.params, rgb, grad_rgb, need=need, residual=res, tex_vd_out=gvd,
-                               dist=dist, grad_dist=grad_dist if ctx.with_dist else None, record=_walk_of(res)), gvd
+                               dist=dist, grad_dist=grad_dist if ctx.with_dist else None, record=_walk_of(res, ctx.scene, ctx.params)), gvd
 
         gs, gsig, gt, gvd = with_room(gradients)
         return gs, gsig, gt, gvd, None, None, None, None, None, None

@@ -110,3 +110,29 @@ def test_gradients_do_not_depend_on_the_room_for_records(monkeypatch, room):
     monkeypatch.setattr(api, "RECORD_BYTES", 8 * n * room)
     got = torch.autograd.grad(sum(api.render(*leaves, o, d, scene, P).square().sum() for o, d in rays), leaves)
     assert all(close(a, b) for a, b in zip(got, want))
+
+
+def test_an_update_between_forward_and_backward():
+    """The backward walks the new sites, with or without room for a record."""
+    sc = W.make_scene("uniform", 2000, 2, 67)
+    rng = np.random.default_rng(68)
+    n = 500
+    d = rng.normal(size=(n, 3))
+    o, d = (torch.as_tensor(x.astype(np.float32), device=DEV)
+            for x in (rng.uniform(0, 1, (n, 3)), d / np.linalg.norm(d, axis=1, keepdims=True)))
+    moved = torch.as_tensor(sc.sites + rng.normal(0, 1e-3, sc.sites.shape).astype(np.float32), device=DEV)
+    P, grads = api.make_params(), []
+    for record in (True, False):
+        scene = api.Scene.from_workload(sc)
+        sigma = torch.as_tensor(sc.sigma, device=DEV).requires_grad_(record)
+        if record:
+            rgb = api.render(torch.as_tensor(sc.sites, device=DEV), sigma, torch.as_tensor(sc.tex, device=DEV), o, d,
+                             scene, P)
+            scene.update(sites=moved)
+            grads.append(torch.autograd.grad(rgb.square().sum(), sigma)[0])
+        else:
+            res = torch.empty(n, 3, device=DEV)
+            rgb = api.render_fwd(scene, o, d, P, residual=res)[0]
+            scene.update(sites=moved)
+            grads.append(api.render_bwd(scene, o, d, P, rgb, 2 * rgb, residual=res)[1])
+    assert close(*grads)

@@ -10,7 +10,7 @@ from paper_2608_17682_gb300 import api  # noqa: E402
 
 
 class StandIn:
-    n, R, has_tex_vd = 4, 2, False
+    n, R, has_tex_vd, updates = 4, 2, False, 0
 
 
 @pytest.fixture
@@ -61,9 +61,9 @@ def test_a_walk_is_recorded_only_for_a_backward(calls, grad_mode, needs):
     assert (calls[0] is not None) == (grad_mode and needs)
 
 
-def render(needs_grad=True):
+def render(scene=None, params=None):
     sites, sigma, tex, o, d = arrays()
-    return api.render(sites, sigma.requires_grad_(needs_grad), tex, o, d, StandIn(), api.make_params())
+    return api.render(sites, sigma.requires_grad_(True), tex, o, d, scene or StandIn(), params or api.make_params())
 
 
 def test_the_record_lives_as_long_as_the_saved_tensors(calls):
@@ -143,3 +143,16 @@ def test_other_failures_stay(calls, monkeypatch, error):
     with pytest.raises((api.VTError, torch.cuda.OutOfMemoryError)):
         render().sum().backward()
     assert len(given) == 1
+
+
+def test_a_changed_scene_or_parameter_leaves_the_record_out(calls, monkeypatch):
+    """The backward walks the scene as it stands, as without a record; timing events are not part of the walk."""
+    scene, params = StandIn(), api.make_params()
+    seen = []
+    for change in (lambda: None, lambda: setattr(scene, "updates", scene.updates + 1),
+                   lambda: setattr(params, "T_eps", 0.5), lambda: params.walk_events.__setitem__(0, 8)):
+        rgb = render(scene, params)
+        change()
+        rgb.sum().backward()
+        seen.append(calls[-1] is not None)
+    assert seen == [True, False, False, True]
