@@ -25,6 +25,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 
 #include "vt.h"
 
@@ -85,10 +86,13 @@ struct vt_scene {
   vt_anchors* anchors = nullptr;
   unsigned long long* anchor_part = nullptr;
   // validation of an update: the device word that its kernels look at, its copy
-  // for the host and the event behind the copy (made by the first update)
+  // for the host, the events behind the copy and behind the last of the kernels
+  // (made by the first update); one update at a time
+  std::mutex update_mu;
   unsigned* bad = nullptr;
   unsigned* host_bad = nullptr;
   cudaEvent_t bad_copied = nullptr;
+  cudaEvent_t bad_read = nullptr;
   // backward scratch: per-cell {dL/ds_x, dL/ds_y, dL/ds_z, dL/dsigma} (twice: even
   // and odd warps' sums), per-texel RGBA
   float4* g_cell = nullptr;

@@ -335,6 +335,7 @@ void free_scene(vt_scene* s) {
   cudaFree(s->bad);
   cudaFreeHost(s->host_bad);
   if (s->bad_copied) cudaEventDestroy(s->bad_copied);
+  if (s->bad_read) cudaEventDestroy(s->bad_read);
   cudaFree(s->rec);
   cudaFree(s->rec_h);
   cudaFree(s->unit);
@@ -530,12 +531,25 @@ vt_status vt_scene_update(vt_scene* s, const float* sites, const float* sigma, c
   // The check of the new values is read back while the kernels that install
   // them are already on their way: they look at its result themselves and
   // change nothing if it refuses. (An allocation and a wait before them had left
-  // the device idle for 40 us of a training step.)
+  // the device idle for 40 us of a training step.) The word that they look at is
+  // the scene's, so an update on another stream waits for them before it uses it.
   const unsigned* bad = nullptr;
+  std::lock_guard<std::mutex> one(s->update_mu);
+  struct Behind {
+    cudaEvent_t event = nullptr;
+    cudaStream_t st = nullptr;
+    ~Behind() {
+      if (event) cudaEventRecord(event, st);
+    }
+  } behind;
   if (sites || sigma) {
     if (!s->bad) VT_CUDA_TRY(cudaMalloc(&s->bad, sizeof(unsigned)));
     if (!s->host_bad) VT_CUDA_TRY(cudaMallocHost(&s->host_bad, sizeof(unsigned)));
     if (!s->bad_copied) VT_CUDA_TRY(cudaEventCreateWithFlags(&s->bad_copied, cudaEventDisableTiming));
+    if (!s->bad_read) VT_CUDA_TRY(cudaEventCreateWithFlags(&s->bad_read, cudaEventDisableTiming));
+    VT_CUDA_TRY(cudaStreamWaitEvent(st, s->bad_read, 0));
+    behind.event = s->bad_read;
+    behind.st = st;
     bad = s->bad;
     const int g = vt_grid(s->n, 256, 152 * 32);
     VT_CUDA_TRY(cudaMemsetAsync(s->bad, 0, sizeof(unsigned), st));

@@ -41,3 +41,27 @@ def test_refused_update_changes_nothing(where, half):
     assert not torch.equal(api.render_fwd(scene, o, d, P)[0], before[0])
     # the graph is the old sites': walks on it are the same in any cell order
     assert torch.equal(api.render_fwd(scene, o, d, P)[0], api.render_fwd(other, o, d, P)[0])
+
+
+def test_a_refused_update_leaves_one_on_another_stream_alone():
+    """An update returns while its kernels run; a refused one on another stream must not stop them half way."""
+    wl = W.make_workload("tiny", n_sites=2000)
+    n, R = 2000, 64  # long rows: the texture pass of the first update is still on its way when the second one is checked
+    scene = api.Scene(wl.scene.sites, wl.scene.sigma, torch.rand(n, R, R, 3, device=DEV), wl.scene.offsets,
+                      wl.scene.indices, tex_vd=torch.rand(n, R, R, 3, device=DEV))
+    o, d = (torch.as_tensor(x, device=DEV) for x in W.workload_rays(wl))
+    P = api.make_params(**wl.params, appearance=1)
+    bad = torch.full((n,), float("nan"), device=DEV)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    for k in range(20):
+        new = [torch.rand(n, 3, device=DEV), torch.rand(n, device=DEV), torch.rand(n, R, R, 3, device=DEV),
+               torch.rand(n, R, R, 3, device=DEV)]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(streams[0]):
+            scene.update(*new)
+        with torch.cuda.stream(streams[1]), pytest.raises(_vt.VTError):
+            scene.update(sigma=bad)
+        torch.cuda.synchronize()
+        got = api.render_fwd(scene, o, d, P)[0]
+        scene.update(*new)
+        assert torch.equal(got, api.render_fwd(scene, o, d, P)[0]), k
