@@ -54,3 +54,29 @@ def test_batch_gradient_is_the_sum_over_its_rays(n, spread, appearance, R):
     for t, w, s in zip(got, want, size):
         assert bool(((t - w).abs() <= (n + 8) * 2.0**-24 * s).all())
     assert scene.get_error()[0] == 0
+
+
+@pytest.mark.parametrize("skip,density", [(2.0, 1.0), (0.0, 0.0)])
+@pytest.mark.parametrize("appearance", [0, 1])
+@pytest.mark.parametrize("order", ["user", "scene"])
+def test_cells_without_colour_take_nothing_of_an_infinite_gradient(skip, density, appearance, order):
+    """No cell is coloured: too little weight for the skip threshold, or no density."""
+    sc = W.make_scene("uniform", 1500, 4, 73)
+    rng = np.random.default_rng(74)
+    n = 200
+    tvd = rng.normal(size=sc.tex.shape).astype(np.float32) if appearance else None
+    sc.sigma[:] *= density
+    scene = api.Scene.from_workload(sc, tex_vd=tvd)
+    d = rng.normal(size=(n, 3))
+    to = torch.as_tensor(rng.uniform(0, 1, (n, 3)).astype(np.float32), device=DEV)
+    td = torch.as_tensor((d / np.linalg.norm(d, axis=1, keepdims=True)).astype(np.float32), device=DEV)
+    g = torch.full((n, 3), float("inf"), device=DEV)
+    P = api.make_params(appearance=appearance, skip_weight=skip)
+    rgb = api.render_fwd(scene, to, td, P)[0]
+    if order == "user":
+        vd = torch.empty(sc.tex.shape, device=DEV) if appearance else None
+        maps = [api.render_bwd(scene, to, td, P, rgb, g, tex_vd_out=vd)[2], vd]
+    else:
+        maps = api.render_bwd_scene_order(scene, to, td, P, rgb, g)[1:]
+    for x in maps:
+        assert x is None or not x.any()
