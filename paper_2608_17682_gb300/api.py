@@ -8,7 +8,6 @@ follows the record and searches only the steps that it does not hold.
 """
 from __future__ import annotations
 
-import collections
 import ctypes
 import threading
 import weakref
@@ -210,26 +209,30 @@ class Walk:
     """A walk record (`record`, None without one) that counts towards RECORD_BYTES
     of its device while it lives, and that with_room may take back."""
 
+    __slots__ = ("record", "key", "_device", "_bytes", "__weakref__")
     _lock = threading.RLock()  # reentrant: a collection within it may end another's life
-    _alive = weakref.WeakSet()
-    _held = collections.Counter()  # bytes per device
+    _held = {}  # bytes per device
+    _alive = {}  # id -> weak reference
 
     def __init__(self, n, device):
-        self.record, device = None, torch.device(device)
+        self.record = None
         if device.type == "cuda" and device.index is None:
             device = torch.device("cuda", torch.cuda.current_device())
-        self._device = device
         with self._lock:
-            self.record = walk_record(n, device, self._held[device])
-            if self.record is not None:
-                self._held[device] += self.record.nbytes
-                self._alive.add(self)
+            held = self._held.get(device, 0)
+            record = walk_record(n, device, held)
+            if record is not None:
+                self.record, self._device, self._bytes = record, device, record.nbytes
+                self._held[device] = held + self._bytes
+                self._alive[id(self)] = weakref.ref(self)
 
     def give_up(self):
-        with self._lock:
-            if self.record is not None:
-                self._held[self._device] -= self.record.nbytes
-                self.record = None
+        if self.record is not None:
+            with self._lock:
+                if self.record is not None:
+                    self.record = None
+                    self._held[self._device] -= self._bytes
+                    del self._alive[id(self)]
 
     __del__ = give_up
 
@@ -243,7 +246,7 @@ def with_room(call):
         if isinstance(e, VTError) and e.status != _vt.VT_ERR_OOM:
             raise
         with Walk._lock:
-            walks = [w for w in Walk._alive if w.record is not None]
+            walks = [w for w in (r() for r in list(Walk._alive.values())) if w is not None]
         if not walks:
             raise
     # (outside the handler, whose exception holds on to the failed call's locals)
@@ -448,16 +451,19 @@ def average_samples_bwd(grad_px, spp):
     return out
 
 
+_PARAM_BYTES = _vt.vt_render_params.walk_events.offset
+
+
 def _walk_key(scene, params):
     """What a walk depends on beside its rays: the scene's values and the render parameters (not their timing events)."""
-    return scene.updates, bytes(params)[:_vt.vt_render_params.walk_events.offset]
+    return scene.updates, bytes(params)[:_PARAM_BYTES]
 
 
 def _walk_of(res, scene, params):
     """The walk record that a saved residual carries, unless the scene or the parameters have changed since: then the
     backward walks the scene as it is."""
     walk = getattr(res, "walk", None)
-    return None if walk is None or res.walk_key != _walk_key(scene, params) else walk.record
+    return walk.record if walk is not None and walk.key == _walk_key(scene, params) else None
 
 
 class VTRender(torch.autograd.Function):
@@ -475,11 +481,11 @@ class VTRender(torch.autograd.Function):
         # The record comes last, what the render needs first. It lives and dies with the saved residual, but is not
         # itself a saved tensor: hooks that pack those (offloading, checkpointing) would move ten times the bytes for
         # what the backward can do without. (grad_mode: it is off in here, and needs_input_grad does not look at it.)
+        walk = None
         if grad_mode and any(ctx.needs_input_grad[:4]):
-            res.walk = Walk(o.shape[0], o.device)
-            res.walk_key = _walk_key(scene, params)
-        render_fwd(scene, o, d, params, out=(rgb, None, None), residual=res, dist=dist,
-                   record=_walk_of(res, scene, params))
+            walk = res.walk = Walk(o.shape[0], o.device)
+            walk.key = _walk_key(scene, params)
+        render_fwd(scene, o, d, params, out=(rgb, None, None), residual=res, dist=dist, record=walk and walk.record)
         ctx.scene, ctx.params, ctx.with_dist = scene, params, with_dist
         ctx.save_for_backward(o, d, rgb, res, dist)
         if with_dist:
