@@ -127,7 +127,7 @@ static inline size_t vt_texel_bytes(int32_t dtype) { return dtype == VT_F32 ? 16
     }                                         \
   } while (0)
 
-// W consecutive floats, 16-byte accesses for W = 4
+// W consecutive floats, a 16-byte access for W = 4
 template <int W>
 struct Chan {
   float x[W];
@@ -150,6 +150,59 @@ __device__ __forceinline__ void store_chan(float* p, const Chan<W>& c) {
   else
     *p = c.x[0];
 }
+
+// a + b = s + e exactly (TwoSum, Knuth)
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// A thread's share of a loss sum: FP32 pairs with error-free sums and products,
+// 48 bits to FP64's 53, as an FP64 operation takes as long as 64 FP32 ones and one
+// per channel costs more than the memory. (Against exact sums of 128 terms, the
+// count of a thread in 1M rays: 1.3e-13 in the worst of 1,024 threads, 6e-15 for
+// their total, which is then rounded to FP32: 6e-8.) What FP32 does not hold goes
+// to an FP64 sum: terms beyond 2^100, infinities and NaN; chunks whose largest
+// number is beyond 2^50 or below 2^-51 (the errors of smaller squares are not FP32
+// numbers; beside a larger square of the chunk they do not count).
+struct LossSum {
+  float hi = 0.f, lo = 0.f;
+  double far = 0.0;
+  __device__ __forceinline__ void add_pair(float x, float xe) {
+    float s, e;
+    two_sum(hi, x, s, e);
+    hi = s;
+    lo = __fadd_rn(lo, __fadd_rn(e, xe));
+  }
+  __device__ __forceinline__ void add(float x) {
+    if (fabsf(x) <= 0x1p100f)
+      add_pair(x, 0.f);
+    else
+      far += (double)x;
+  }
+  template <int W>
+  __device__ __forceinline__ void add_squares(const Chan<W>& r) {
+    bool near = true;
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      near = near && fabsf(r.x[i]) <= 0x1p50f;  // (false for NaN)
+      m = fmaxf(m, fabsf(r.x[i]));
+    }
+    if (near && (m >= 0x1p-51f || m == 0.f)) {
+#pragma unroll
+      for (int i = 0; i < W; ++i) {
+        const float p = __fmul_rn(r.x[i], r.x[i]);
+        add_pair(p, __fmaf_rn(r.x[i], r.x[i], -p));
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < W; ++i) far += (double)r.x[i] * (double)r.x[i];
+    }
+  }
+  __device__ __forceinline__ double total() const { return far + ((double)hi + (double)lo); }
+};
 
 static inline int vt_grid(int64_t n, int block, int64_t cap = 1 << 30) {
   int64_t g = (n + block - 1) / block;

@@ -102,3 +102,51 @@ def test_gradient_rows_in_user_order(R):
         for a, b in ((gt[perm], tex[..., :3]), (again[perm], tex[..., :3]), (gs[perm], cell[:, :3]),
                      (gsig[perm], cell[:, 3])):
             assert (a - b).abs().max() <= 1e-4 * b.abs().max()
+
+
+# The losses' sums hold what FP64 sums of the channels hold: bits that an FP32 sum of a chunk or row loses (small terms
+# beside a large one), and squares beyond FP32's range. The results are FP32: one rounding each of the mean's factor and
+# of the sum, 2^-24 each, the mean's where there are several blocks a few more.
+BITS = 2.2 * 2.0**-24
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("far", [False, True])
+def test_loss_sums_keep_what_fp64_holds(far, shift):
+    n = 1024
+    r = np.full((n, 3), 0.99 * 2.0**-12, np.float32)
+    r.reshape(-1)[::4] = 1.0
+    if far:  # 1e40 / 3072 is an FP32 number, 1e40 is not
+        r[700, 1] = -1e20
+    tr, zero = at(r, shift), at(np.zeros((n, 3), np.float32), shift)
+    r, loss = r.astype(np.float64), torch.empty(1, device=DEV)
+    _vt.vt_l2_loss(n, tr.data_ptr(), zero.data_ptr(), 0, loss.data_ptr(), api._stream())
+    assert abs(loss.item() - (r * r).mean()) <= BITS * (r * r).mean()
+    _vt.vt_smooth_l1_loss(n, tr.data_ptr(), zero.data_ptr(), 2.0, 0, loss.data_ptr(), api._stream())
+    L = TR.smooth_l1(r, 0 * r, 2.0)[0]  # its terms are FP32: half an ulp each
+    assert abs(loss.item() - L) <= (BITS + 2.0**-24) * L
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("scale,lam", [(1.0, 1.0), (1e25, 1e-22), (1e-25, 1e32)])
+@pytest.mark.parametrize("R", [2, 7, 8, 64])
+def test_regulariser_sums_keep_what_fp64_holds(R, scale, lam, shift):
+    """One cell, so one block. A row's first channels are large, the mean of each colour is zero."""
+    p = np.full((1, R * R, 3), 2.0**-13, np.float32)
+    p[0, 1::2] *= -1
+    if R % 2:
+        p[0, -1] = 0.0
+    p[0, 0], p[0, 1] = 1.0, -1.0
+    p = (p * np.float32(scale)).reshape(1, R, R, 3)
+    tp, z = at(p, shift), torch.zeros(1, dtype=torch.int32, device=DEV)
+    loss = torch.zeros(1, device=DEV)
+    want = {0: TR.texture_regularizers(p, 0 * p, 0.0, lam)[0], 1: TR.texture_regularizers(0 * p, p, lam, 0.0)[0]}
+    for reg in (0, 1):
+        loss.zero_()
+        _vt.vt_adam_step_tex_scene_order(1, R, z.data_ptr(), 0, tp.data_ptr(), 0, 0, reg, lam, 0.0, 0.9, 0.999, 1e-15, 1,
+                                         loss.data_ptr(), api._stream())
+        # besides: the weight and 1/R^2 in FP32, and in reg 0 the deviations from an FP32 mean of 2^-24 or so
+        assert abs(loss.item() - want[reg]) <= 2 * BITS * want[reg]
+        args = (tp.data_ptr(), 0, 0.0, lam) if reg == 0 else (0, tp.data_ptr(), lam, 0.0)
+        _vt.vt_texture_regularizers(1, R, *args, 0, 0, loss.data_ptr(), api._stream())
+        assert abs(loss.item() - want[reg]) <= 2 * BITS * want[reg]
