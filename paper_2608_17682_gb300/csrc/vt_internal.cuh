@@ -139,7 +139,8 @@ __device__ __forceinline__ Chan<W> load_chan(const float* p) {
     const float4 q = *reinterpret_cast<const float4*>(p);
     c.x[0] = q.x, c.x[1] = q.y, c.x[2] = q.z, c.x[3] = q.w;
   } else {
-    c.x[0] = *p;
+#pragma unroll
+    for (int i = 0; i < W; ++i) c.x[i] = p[i];
   }
   return c;
 }
@@ -148,7 +149,8 @@ __device__ __forceinline__ void store_chan(float* p, const Chan<W>& c) {
   if constexpr (W == 4)
     *reinterpret_cast<float4*>(p) = make_float4(c.x[0], c.x[1], c.x[2], c.x[3]);
   else
-    *p = c.x[0];
+#pragma unroll
+    for (int i = 0; i < W; ++i) p[i] = c.x[i];
 }
 
 // a + b = s + e exactly (TwoSum, Knuth)
