@@ -59,3 +59,48 @@ def test_small_launches_equal_a_large_one(appearance, with_dist, dtype):
     for k, x in enumerate(whole):
         assert torch.equal(torch.cat([p[k] for p in parts]), x)
     assert scene.get_error()[0] == 0
+
+
+def lattice_scene(k, seed):
+    """Sites of a cubic lattice, moved by a few FP32 roundings, with all 26 neighbours: cells meet eight in a corner."""
+    rng = np.random.default_rng(seed)
+    at = np.arange(k)
+    ijk = np.stack(np.meshgrid(at, at, at, indexing="ij"), -1).reshape(-1, 3)
+    sites = (ijk / k + rng.uniform(-2e-7, 2e-7, ijk.shape)).astype(np.float32)
+    rows = []
+    for c in ijk:
+        lo, hi = np.maximum(c - 1, 0), np.minimum(c + 2, k)
+        n = np.stack(np.meshgrid(*(np.arange(a, b) for a, b in zip(lo, hi)), indexing="ij"), -1).reshape(-1, 3)
+        n = n[(n != c).any(1)]
+        rows.append(rng.permutation((n[:, 0] * k + n[:, 1]) * k + n[:, 2]))
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
+    n = len(sites)
+    return W.Scene(sites, np.exp(rng.normal(-1, 1, n)).astype(np.float32), W.textures(n, 2, rng), off.astype(np.int64),
+                   np.concatenate(rows).astype(np.int32))
+
+
+def test_teams_take_the_same_of_planes_equal_within_rounding():
+    """Rays through corners: seven crossings within some roundings of one another, whose comparisons depend on their
+    order. The walk's cells and steps must be the single lane's."""
+    k, n = 8, 120_000
+    sc = lattice_scene(k, 83)
+    rng = np.random.default_rng(84)
+    corner = (rng.integers(1, k - 2, (n, 3)) + 0.5) / k
+    d = rng.normal(size=(n, 3))
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    o = corner - rng.uniform(0.02, 0.5, (n, 1)) * d
+    scene = api.Scene.from_workload(sc)
+    to, td = (torch.as_tensor(x.astype(np.float32), device=DEV) for x in (o, d))
+    P = api.make_params(T_eps=0.0)
+
+    def walk(a, b):
+        rec = torch.zeros(40, b - a, dtype=torch.int64, device=DEV)
+        out = api.render_fwd(scene, to[a:b], td[a:b], P, record=rec)
+        return [*out, rec.t().contiguous()]
+
+    whole = walk(0, n)
+    parts = [walk(a, a + 20_000) for a in range(0, n, 20_000)]
+    differ = [int((torch.cat([p[i] for p in parts]) != x).reshape(n, -1).any(1).sum()) for i, x in enumerate(whole)]
+    assert differ == [0, 0, 0, 0]
+    single = api.trace_cells(scene, to[:20_000], td[:20_000], P, max_cells=32)  # (a lane per ray at any size)
+    assert torch.equal(single[2], parts[0][2])
