@@ -80,3 +80,34 @@ def test_cells_without_colour_take_nothing_of_an_infinite_gradient(skip, density
         maps = api.render_bwd_scene_order(scene, to, td, P, rgb, g)[1:]
     for x in maps:
         assert x is None or not x.any()
+
+
+def test_cell_sums_of_a_scene_of_more_than_32_bits_of_texels():
+    """A row of 2^20 + 1 slabs with 64x64 textures (110 GB). 2^26 times the same ray: a running FP32 sum of the rays'
+    density gradients, in an array each for odd and even warps, stops growing at 2^24 addends; one of whole warps' sums,
+    2^20 each, is off by 2^20 roundings of 2^-25 at most."""
+    free = torch.cuda.mem_get_info()[0]
+    if free < 140 << 30:
+        pytest.skip("needs 140 GB of device memory")
+    n, R, rays = (1 << 20) + 1, 64, 1 << 26
+    x = torch.arange(n, device=DEV)
+    sites = torch.stack([x.float(), 0 * x.float(), 0 * x.float()], 1)
+    off = torch.clamp(2 * torch.arange(n + 1, device=DEV) - 1, 0, 2 * (n - 1))
+    idx = torch.stack([x - 1, x + 1], 1).reshape(-1)
+    idx = idx[(idx >= 0) & (idx < n)].int()
+    tex = torch.zeros(n, R, R, 3, device=DEV)
+    scene = api.Scene(sites, torch.full((n,), 3.0, device=DEV), tex, off, idx, tex_dtype="f16")
+    del tex, x
+    torch.cuda.empty_cache()
+    P = api.make_params(skip_weight=2.0)  # no colours: the background shines through
+    to = torch.tensor([[777_000.1, 0.0, 0.0]], device=DEV).repeat(rays, 1)
+    td = torch.tensor([[1.0, 0.0, 0.0]], device=DEV).repeat(rays, 1)
+    rgb = api.render_fwd(scene, to, td, P, want_steps=False)[0]
+
+    def density_gradient(k):
+        return api.render_bwd(scene, to[:k], td[:k], P, rgb[:k], torch.ones(k, 3, device=DEV), need=(True, True, False))[1]
+
+    one, all_ = density_gradient(1).double(), density_gradient(rays).double()
+    assert int((one != 0).sum()) > 1
+    assert bool(((all_ - rays * one).abs() <= rays * (one.abs() * 2.0**20 * 2.0**-25)).all())
+    scene.close()
