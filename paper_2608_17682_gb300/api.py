@@ -185,18 +185,20 @@ def generate_rays(cameras, device="cuda", out=None):
 
 
 # A walk record holds up to RECORD_STEPS steps of every ray (the rays of the
-# surface scenes take 7 to 19 cells on average, 60 at most), fewer where the
-# records alive on a device would pass RECORD_BYTES together; what a record does
-# not hold is searched again.
+# surface scenes take 7 to 19 cells on average, 60 at most), fewer where it
+# would pass RECORD_BYTES, or with the others alive on the device
+# ALL_RECORDS_BYTES (ten 1280x832 views, or as many trainers of 2^20 rays a step);
+# what a record does not hold is searched again.
 RECORD_STEPS = 48
 RECORD_BYTES = 1 << 30
+ALL_RECORDS_BYTES = 4 << 30
 
 
 def walk_record(n, device, held=0):
     """Memory for render_fwd(record=) of n rays: int64 [steps + 2, n] (8 bytes
-    per step, opaque), or None where it would hold less than 8 steps within
-    RECORD_BYTES less `held` bytes, or the device has no room for it."""
-    steps = min(RECORD_STEPS, (RECORD_BYTES - held) // (8 * n) - 2) if n else 0
+    per step, opaque), or None where it would hold less than 8 steps within the
+    bounds (`held`: bytes of other records), or the device has no room for it."""
+    steps = min(RECORD_STEPS, min(RECORD_BYTES, ALL_RECORDS_BYTES - held) // (8 * n) - 2) if n else 0
     if steps < 8:
         return None
     try:
@@ -206,8 +208,9 @@ def walk_record(n, device, held=0):
 
 
 class Walk:
-    """A walk record (`record`, None without one) that counts towards RECORD_BYTES
-    of its device while it lives, and that with_room may take back."""
+    """A walk record (`record`, None without one) that counts towards
+    ALL_RECORDS_BYTES of its device while it lives, and that with_room may take
+    back."""
 
     __slots__ = ("record", "key", "_device", "_bytes", "__weakref__")
     _lock = threading.RLock()  # reentrant: a collection within it may end another's life

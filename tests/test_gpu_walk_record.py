@@ -107,7 +107,8 @@ def test_gradients_do_not_depend_on_the_room_for_records(monkeypatch, room):
     monkeypatch.setattr(api, "RECORD_BYTES", 0)
     want = [sum(g) for g in zip(*(torch.autograd.grad(api.render(*leaves, o, d, scene, P).square().sum(), leaves)
                                   for o, d in rays))]
-    monkeypatch.setattr(api, "RECORD_BYTES", 8 * n * room)
+    monkeypatch.undo()
+    monkeypatch.setattr(api, "ALL_RECORDS_BYTES", 8 * n * room)
     got = torch.autograd.grad(sum(api.render(*leaves, o, d, scene, P).square().sum() for o, d in rays), leaves)
     assert all(close(a, b) for a, b in zip(got, want))
 

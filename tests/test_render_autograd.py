@@ -92,10 +92,11 @@ STEP = 8 * 16  # bytes of a step of the stand-in's 16 rays
 
 
 def test_renders_that_live_together_share_the_bound(calls, monkeypatch):
-    monkeypatch.setattr(api, "RECORD_BYTES", STEP * (api.RECORD_STEPS + 2 + 30) + 1)
+    monkeypatch.setattr(api, "RECORD_BYTES", STEP * 40)
+    monkeypatch.setattr(api, "ALL_RECORDS_BYTES", STEP * (40 + 40 + 30) + 1)
     for _ in range(2):  # what the first round held is given back
-        alive = [render() for _ in range(4)]
-        assert [r and r().shape[0] for r in calls] == [api.RECORD_STEPS + 2, 30, None, None]
+        alive = [render() for _ in range(5)]
+        assert [r and r().shape[0] for r in calls] == [40, 40, 30, None, None]
         sum(x.sum() for x in alive).backward()
         del calls[:], alive
 
