@@ -162,9 +162,9 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 
 // A thread's share of a loss sum: FP32 pairs with error-free sums and products,
 // 48 bits to FP64's 53, as an FP64 operation takes as long as 64 FP32 ones and one
-// per channel costs more than the memory. (Against exact sums of 128 terms, the
-// count of a thread in 1M rays: 1.3e-13 in the worst of 1,024 threads, 6e-15 for
-// their total, which is then rounded to FP32: 6e-8.) What FP32 does not hold goes
+// per channel costs more than the memory. (Against exact sums of squares, worst of
+// uniform, normal and log-normal terms: 1.2e-13 of 128, 1e-12 of 4,096; the losses
+// are then rounded to FP32, 6e-8.) What FP32 does not hold goes
 // to an FP64 sum: terms beyond 2^100, infinities and NaN; chunks whose largest
 // number is beyond 2^50 or below 2^-51 (the errors of smaller squares are not FP32
 // numbers; beside a larger square of the chunk they do not count).
@@ -183,16 +183,26 @@ struct LossSum {
     else
       far += (double)x;
   }
+  // Where a chunk's squares are at most the sum so far, hi - s below is exact
+  // (s <= 2 hi): one rounding each of a square's sum and of that sum's error.
   template <int W>
   __device__ __forceinline__ void add_squares(const Chan<W>& r) {
-    bool near = true;
     float m = 0.f;
 #pragma unroll
-    for (int i = 0; i < W; ++i) {
-      near = near && fabsf(r.x[i]) <= 0x1p50f;  // (false for NaN)
-      m = fmaxf(m, fabsf(r.x[i]));
+    for (int i = 0; i < W; ++i) m = fmaxf(m, fabsf(r.x[i]));
+    if (__fmul_rn(m, m) <= hi && hi >= 0x1p-100f && hi <= 0x1p110f) {  // (a NaN in r makes hi one)
+#pragma unroll
+      for (int i = 0; i < W; ++i) {
+        const float s = __fmaf_rn(r.x[i], r.x[i], hi);
+        lo = __fadd_rn(lo, __fmaf_rn(r.x[i], r.x[i], __fsub_rn(hi, s)));
+        hi = s;
+      }
+      return;
     }
-    if (near && (m >= 0x1p-51f || m == 0.f)) {
+    bool near = m >= 0x1p-51f || m == 0.f;
+#pragma unroll
+    for (int i = 0; i < W; ++i) near = near && fabsf(r.x[i]) <= 0x1p50f;  // (false for NaN)
+    if (near) {
 #pragma unroll
       for (int i = 0; i < W; ++i) {
         const float p = __fmul_rn(r.x[i], r.x[i]);
