@@ -285,7 +285,8 @@ vt_status vt_render_bwd(vt_scene* s, int64_t n_rays, const float* o, const float
  * the record are searched. Results are those of vt_render_fwd and vt_render_bwd
  * (the backward's sums in another order). The caller owns the record, which must
  * be the one that vt_render_fwd_record wrote for the same scene, rays and
- * parameters. record NULL: none is written, or the backward searches. */
+ * parameters; VT_ERR_INVALID_ARG if it is not 8-byte aligned or record_steps is
+ * negative. record NULL: none is written, or the backward searches. */
 vt_status vt_render_fwd_record(vt_scene* s, int64_t n_rays, const float* o, const float* d, const float* time,
                                const vt_render_params* p, float* rgb_out, float* T_out, int32_t* steps_out,
                                float* rgb_residual, float* dist_out, void* record, int32_t record_steps,

@@ -77,6 +77,21 @@ def test_host_argument_validation(vt):
     assert vt.lib.vt_average_samples(4, 0, None, None, None) == vt.VT_ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("record,steps", [(12, 4), (9, 0), (16, -1)])
+def test_walk_record_arguments(vt, record, steps):
+    """A record that is not 8-byte aligned, or of negative length, is refused before anything is read through a
+    pointer (the scene here is not one)."""
+    import ctypes as C
+    p = vt.vt_render_params_default()
+    a, b = C.c_void_p(), C.c_void_p()
+    assert vt.lib.vt_render_fwd_record(8, 0, 8, 8, None, C.byref(p), 8, None, None, None, None, record, steps,
+                                       None) == vt.VT_ERR_INVALID_ARG
+    assert vt.lib.vt_render_bwd_recorded(8, 0, 8, 8, None, C.byref(p), 8, None, None, 8, None, record, steps, None, None,
+                                         None, None, None) == vt.VT_ERR_INVALID_ARG
+    assert vt.lib.vt_render_bwd_scene_order_recorded(8, 0, 8, 8, None, C.byref(p), 8, None, None, 8, None, record, steps,
+                                                     C.byref(a), C.byref(b), None, None) == vt.VT_ERR_INVALID_ARG
+
+
 def test_workload_csr_is_a_valid_delaunay_graph():
     from paper_2608_17682_gb300 import workloads as W
     sc = W.make_scene("uniform", 3000, 4, 5)
