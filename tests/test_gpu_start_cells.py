@@ -58,3 +58,46 @@ def test_start_cells_of_a_batch_laid_out_as_images(cloud, cams):
     oc, _, _, flags = O.trace(osc, eyes[which], d, max_cells=64, params=O.make_params())
     ok = (flags & O.BAND_FLAGS) == 0
     assert np.array_equal(cells.cpu().numpy()[ok], oc[ok])
+
+
+@pytest.mark.parametrize("far", [0.0, 3.0, 1e4, 1e19])
+def test_descent_among_equal_distances(far):
+    """Lattice sites, all 26 neighbours: origins at cell corners, edges and faces have two to eight nearest sites, of
+    which the lowest id counts. `far`: origins that far outside, whose distances FP32 hardly or no longer tells apart;
+    there the cell's own key must be the least among its neighbours'."""
+    k, n = 7, 5000
+    ijk = np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    rng = np.random.default_rng(91)
+    ids = rng.permutation(k**3)  # site of each lattice place
+    step = np.array([s for s in np.ndindex(3, 3, 3) if s != (1, 1, 1)]) - 1
+    rows = [None] * k**3
+    for place, at in enumerate(ijk):
+        nb = at + step
+        nb = nb[((nb >= 0) & (nb < k)).all(1)]
+        rows[ids[place]] = ids[(nb * [k * k, k, 1]).sum(1)]
+    sites = np.empty((k**3, 3), np.float32)
+    sites[ids] = ijk
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    sc = W.Scene(sites, np.ones(k**3, np.float32), W.textures(k**3, 2, rng), off, np.concatenate(rows).astype(np.int32))
+    scene = api.Scene.from_workload(sc)
+    o = (0.5 * rng.integers(0, 2 * k - 1, (n, 3))).astype(np.float32)
+    d = rng.normal(size=(n, 3))
+    d = (d / np.linalg.norm(d, axis=1, keepdims=True)).astype(np.float32)
+    o = o + np.float32(far) * np.sign(d) * (rng.random((n, 3)) < 0.5).astype(np.float32)
+    cells = api.trace_cells(scene, torch.as_tensor(o, device=DEV), torch.as_tensor(d, device=DEV), api.make_params(),
+                            max_cells=1)[0][:, 0].cpu().numpy()
+    with np.errstate(over="ignore"):
+        if far <= 3.0:  # exact in FP32
+            d2 = ((o[:, None] - sites) ** 2).sum(2)
+            assert np.array_equal(cells, d2.argmin(1))  # the first, so the lowest id
+            return
+        delta = np.float32(o[:, None] - sites).astype(np.float64)
+
+        def key(i, j):  # FP32 distance as the kernel forms it: products and sums rounded once each
+            x, y, z = delta[i, j]
+            t = np.float32(z * z).astype(np.float64)
+            t = np.float32(y * y + t).astype(np.float64)
+            return float(np.float32(x * x + t)), j
+
+        for i in range(0, n, 10):
+            assert key(i, cells[i]) <= min(key(i, j) for j in rows[cells[i]])
