@@ -1,6 +1,6 @@
 """Start cells of 1-D batches: batch sizes around the anchors' strides, with one
-origin, a few (kept by the fine anchors, rays match another anchor's origin),
-just more than a few and all different (coarse anchors and greedy descents)."""
+origin, some (fine anchors, rays match another anchor's origin), up to and beyond
+half the anchors, and all different (coarse anchors and greedy descents)."""
 import numpy as np
 import pytest
 
@@ -24,7 +24,7 @@ def cloud():
 
 
 @pytest.mark.parametrize("n", [1, 63, 64, 65, 4096, 4097, 9001, 270_001])
-@pytest.mark.parametrize("origins", [1, 4, 9, 0])
+@pytest.mark.parametrize("origins", [1, 4, 9, 30, 40, 0])
 def test_start_cells_of_a_batch(cloud, n, origins):
     osc, scene = cloud
     rng = np.random.default_rng(n + 7 * origins)
