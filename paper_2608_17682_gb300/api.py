@@ -513,5 +513,9 @@ class VTRender(torch.autograd.Function):
 
 def render(sites, sigma, tex, o, d, scene: Scene, params, tex_vd=None, with_dist=False):
     """Differentiable render; returns rgb, or (rgb, L_dist per ray) with
-    with_dist=True (distortion loss of Sec. 5.3, Eq. 2)."""
+    with_dist=True (distortion loss of Sec. 5.3, Eq. 2). Where a backward can come,
+    the forward's walk is recorded for it within RECORD_BYTES and
+    ALL_RECORDS_BYTES; the memory is released with the graph's saved tensors, or
+    before where the device has none left for a backward. After an update of the
+    scene the backward walks the scene as it is then."""
     return VTRender.apply(sites, sigma, tex, tex_vd, o, d, scene, params, with_dist, torch.is_grad_enabled())

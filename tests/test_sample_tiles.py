@@ -42,6 +42,9 @@ def test_rows_of_samples_follow_image_rows(sizes, frac):
 
 def test_no_layout_for_sparse_samples_or_many_cameras():
     assert train.sample_tiles(cams(4, 100, 100), 4000) is None  # 10 samples a row
-    assert train.sample_tiles(cams(40, 63, 64), 40 * 63 * 64 - 100) is None or \
-        len(train.sample_tiles(cams(40, 63, 64), 40 * 63 * 64 - 100)) <= 64
+    # 4,029 samples of each camera: 63 rows of 63 and 60 more, two images each
+    for n in (31, 32):
+        tiles = train.sample_tiles(cams(n, 63, 64), n * 4029)
+        assert tiles == [(63, 63), (60, 1)] * n
+    assert train.sample_tiles(cams(33, 63, 64), 33 * 4029) is None
     assert train.sample_tiles(cams(70, 64, 64), 70 * 64 * 64) is None
