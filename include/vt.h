@@ -152,8 +152,9 @@ vt_status vt_scene_create(const vt_scene_desc* desc, void* stream, vt_scene** ou
  * N, R and adjacency as at creation; any may be NULL to keep the old one;
  * tex_vd only if the scene was created with one). The Morton order of
  * creation is kept. Validates like vt_scene_create: waits for the check on
- * `stream`, not for the copies, and leaves the scene as it was if it refuses.
- * Updates of one scene are taken one at a time, on any streams; renders on other
+ * `stream`, not for the copies, and leaves the scene as it was if it refuses
+ * (with VT_SCENE_HALF_OFFSETS, offsets out of range are only found when the new
+ * values are in). Updates of one scene are taken one at a time, on any streams; renders on other
  * streams than an update's are the caller's to order. */
 vt_status vt_scene_update(vt_scene* s, const float* sites, const float* sigma, const float* tex,
                           const float* tex_vd, void* stream);

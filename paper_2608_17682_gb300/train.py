@@ -166,6 +166,7 @@ class Trainer:
         self.refreshes += 1
 
     # ------------------------------------------------------------------ one iteration
+    @property
     def step_params(self):
         """The render parameters as they stand, with the samples' launch layout unless they have their own."""
         p, t = self.rparams, self.tiles
@@ -178,7 +179,7 @@ class Trainer:
     def step(self, sync_loss=False):
         cfg, s = self.cfg, _vt
         st = api._stream()
-        params = self.step_params()
+        params = self.step_params
         if self.it > 0 and cfg.refresh_every > 0 and self.it % cfg.refresh_every == 0:
             self.refresh()
         _vt.vt_sigma_from_rho(self.sigma.numel(), self.p["rho"].data_ptr(), self.sigma.data_ptr(), st)

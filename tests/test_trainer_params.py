@@ -37,14 +37,14 @@ def trainer(monkeypatch):
 
 @pytest.mark.parametrize("rp", [{}, {"image_sizes": None}, {"img_w": 0, "img_h": 0, "n_images": 0}, {"n_images": 1}])
 def test_parameters_without_a_layout(trainer, rp):
-    p = trainer(t_far=7.0, **rp).step_params()
+    p = trainer(t_far=7.0, **rp).step_params
     assert (p.t_far, p.appearance, p.n_images, bool(p.image_sizes)) == (7.0, 1, 2, True)
 
 
 @pytest.mark.parametrize("rp", [{"img_w": 64, "img_h": 48, "n_images": 2}, {"image_sizes": [(64, 96)]}])
 def test_the_callers_layout_stays(trainer, rp):
     t = trainer(**rp)
-    p = t.step_params()
+    p = t.step_params
     assert (p.img_w, p.image_sizes, p.n_images) == (t.rparams.img_w, t.rparams.image_sizes, rp.get("n_images", 1))
 
 
@@ -58,4 +58,4 @@ def test_the_record_counts_while_the_trainer_lives(trainer):
 def test_later_changes_reach_the_steps(trainer):
     t = trainer()
     t.rparams.T_eps = 0.25
-    assert t.step_params().T_eps == 0.25 and t.step_params().image_sizes and not t.rparams.image_sizes
+    assert t.step_params.T_eps == 0.25 and t.step_params.image_sizes and not t.rparams.image_sizes
