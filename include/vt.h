@@ -154,8 +154,8 @@ vt_status vt_scene_create(const vt_scene_desc* desc, void* stream, vt_scene** ou
  * creation is kept. Validates like vt_scene_create: waits for the check on
  * `stream`, not for the copies, and leaves the scene as it was if it refuses
  * (with VT_SCENE_HALF_OFFSETS, offsets out of range are only found when the new
- * values are in). Updates of one scene are taken one at a time, on any streams; renders on other
- * streams than an update's are the caller's to order. */
+ * values are in). Updates of one scene are taken one at a time, on any streams;
+ * renders on other streams than an update's are the caller's to order. */
 vt_status vt_scene_update(vt_scene* s, const float* sites, const float* sigma, const float* tex,
                           const float* tex_vd, void* stream);
 
