@@ -64,8 +64,9 @@ def test_recorded_backward_matches_the_searching_one(steps, appearance, with_dis
     assert scene.get_error()[0] == 0
 
 
+@pytest.mark.parametrize("layout", [{}, {"image_sizes": [(25, 12), (20, 10)]}])
 @pytest.mark.parametrize("steps", [0, 3, 4, 5, 20])
-def test_record_of_rays_stopped_by_max_steps(steps):
+def test_record_of_rays_stopped_by_max_steps(steps, layout):
     sc = W.make_scene("uniform", 2000, 2, 63)
     scene = api.Scene.from_workload(sc)
     rng = np.random.default_rng(64)
@@ -73,7 +74,7 @@ def test_record_of_rays_stopped_by_max_steps(steps):
     to = torch.as_tensor(rng.uniform(0.3, 0.7, (n, 3)).astype(np.float32), device=DEV)
     d = rng.normal(size=(n, 3))
     td = torch.as_tensor((d / np.linalg.norm(d, axis=1, keepdims=True)).astype(np.float32), device=DEV)
-    P = api.make_params(T_eps=0.0, max_steps=4)
+    P = api.make_params(T_eps=0.0, max_steps=4, **layout)
     rec = torch.full((steps + 2, n), -2, dtype=torch.int64, device=DEV)
     rgb = api.render_fwd(scene, to, td, P, record=rec)[0]
     g = torch.as_tensor(rng.normal(size=(n, 3)).astype(np.float32), device=DEV)
